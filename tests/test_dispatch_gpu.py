@@ -322,3 +322,24 @@ def test_one_channel_weight_gradients_keep_float32(shape, batch):
             ref = np.asarray(grads[layer][k], np.float64).reshape(sh)
             d = np.abs(got[off:off + ref.size].reshape(sh) - ref)
             assert (d <= 64 * 2.0 ** -22 * np.asarray(mags[k]).reshape(sh)).all(), (layer, k, d.max())
+
+
+@pytest.mark.parametrize("nr,L", [(3, 0), (33, 8)])
+def test_render_transpose_keeps_small_partial_sums(nr, L):
+    """A shell's sum over 256 angles: seven of eight runs of 32 sum to 0.45 ulp
+    of the first's, so that adding them to it one by one in float32 loses 3
+    ulps. Within a run the terms are equal and their sums exact, so what
+    remains is each product's rounding and the last one: 2^-23 of the value."""
+    from paper_2608_16960_gb300.model import ShellSH
+    e = synth.grid_edges(nr, 16, 16)
+    m = ShellSH(e, L)
+    y0 = m.tables()[1][0]
+    assert (y0 == y0[0]).all()
+    small = 0.45 * np.spacing(np.float32(32) * y0[0]) / (32 * y0[0])
+    g = np.full((nr, 256), small, np.float32)
+    g[:, :32] = 1.0
+    c = torch.zeros(m.coeff_shape, device="cuda", requires_grad=True)
+    m.render(c).backward(torch.tensor(g.reshape(nr, 16, 16), device="cuda"))
+    got = c.grad[:, 0].double().cpu().numpy()
+    ref = (g.astype(np.float64) * np.float64(y0[0])).sum(1)
+    assert (np.abs(got - ref) <= 2.0 ** -23 * ref).all(), (got - ref) / ref
