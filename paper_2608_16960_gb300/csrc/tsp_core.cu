@@ -134,8 +134,18 @@ extern "C" tsp_status tsp_grid_create(const double* r_edges, int n_r_edges, cons
   g->r.assign(r_edges, r_edges + n_r_edges);
   g->th.assign(theta_edges, theta_edges + n_theta_edges);
   g->ph.assign(phi_edges, phi_edges + n_phi_edges);
+  // The walk runs in a unit in which the outer radius is 2^30 to 2^31: its roots
+  // and quotients take squared lengths below 1.2e-38 for zero, and a line aimed at
+  // the origin passes it at the rounding residue of its float-float set-up, down
+  // to 2^-72 of the start's distance (squared, 1e-41 for a start at 60; such a
+  // line lost the jump of its polar index at the origin).
+  std::vector<double> radii(g->r);
+  const int k = std::min(126, std::max(-126, 30 - std::ilogb(radii.back())));
+  for (double& r : radii) r = std::ldexp(r, k);
+  g->scale = std::ldexp(1.0f, k);
+  g->unit = std::ldexp(1.0f, -k);
   std::vector<float> table;
-  tsp::build_grid_table(r_edges, n_r_edges, theta_edges, n_theta_edges, phi_edges, n_phi_edges, &table, g);
+  tsp::build_grid_table(radii.data(), n_r_edges, theta_edges, n_theta_edges, phi_edges, n_phi_edges, &table, g);
   // Kernels stage the table in shared memory beside the cone lists (24 KB a
   // block): at most 227 KB a block on this GPU. The grid limits keep the table
   // under 107 KB, so this only guards the layout's arithmetic.

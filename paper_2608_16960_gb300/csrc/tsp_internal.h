@@ -21,6 +21,7 @@ struct tsp_grid_s {
   float* d_centres = nullptr;  // voxel centres: r [Nr] | sin t [Ne] | cos t [Ne] | cos p [Na] | sin p [Na]
   int device = 0;
   std::vector<double> r, th, ph;
+  float scale = 1.0f, unit = 1.0f;  // of the table (GridDesc)
   tsp::GridDesc desc() const {
     tsp::GridDesc d;
     d.table = d_table;
@@ -30,6 +31,8 @@ struct tsp_grid_s {
     d.M = M;
     d.words = words;
     d.pa0 = pa0;
+    d.scale = scale;
+    d.unit = unit;
     return d;
   }
   int64_t voxels() const { return int64_t(Nr) * Ne * Na; }

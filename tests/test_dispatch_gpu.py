@@ -343,3 +343,37 @@ def test_render_transpose_keeps_small_partial_sums(nr, L):
     got = c.grad[:, 0].double().cpu().numpy()
     ref = (g.astype(np.float64) * np.float64(y0[0])).sum(1)
     assert (np.abs(got - ref) <= 2.0 ** -23 * ref).all(), (got - ref) / ref
+
+
+@pytest.mark.parametrize("kind", ["cone", "parallel"])
+def test_rays_aimed_at_the_origin(kind):
+    """The centre pixel of an odd detector: the line passes the origin at the
+    rounding residue of its set-up, anywhere from zero to 1e-13, and its polar
+    and azimuth indices jump there, inside the innermost sphere. Each ray within
+    the parity rule of the oracle's."""
+    import oracle
+    from _util import parity
+    grid, e = _grid((20, 16, 31))
+    pos = [synth.random_positions(400, 5)]
+    pos += [synth.circular_orbit(1000, 60.0, incline_deg=a, phase=0.3) for a in (1.0, 5.0, 20.0)]
+    pos = np.concatenate(pos)
+    rho = synth.uniform_volume(grid.shape, 3, 0.1, 1.0)
+    if kind == "cone":
+        geom, rays = Geometry.cone(pos, (1, 1), 5.0), oracle.cone_rays(pos, 1, 1, 5.0)
+    else:
+        geom, rays = Geometry.parallel(pos, (1, 1), 5.0), oracle.parallel_rays(pos, 1, 1, 5.0)
+    y = tsp_forward(grid, geom, torch.tensor(rho, device="cuda")).cpu().numpy()
+    parity(y, oracle.forward(e, *rays, rho), what=f"{kind} rays aimed at the origin")
+
+
+@pytest.mark.parametrize("k", [-60, -20, 7, 40])
+def test_units_of_length(k):
+    """Grid and views in a unit 2^-k times the other's: the same lengths times
+    2^k, exactly (a grid whose squared radii approach the smallest floats too)."""
+    e = synth.grid_edges(20, 15, 30)
+    pos = synth.circular_orbit(3, 60.0, incline_deg=20.0, phase=0.3)
+    rho = torch.tensor(synth.uniform_volume((20, 15, 30), 3, 0.1, 1.0), device="cuda")
+    a = tsp_forward(Grid.from_edges(e), Geometry.cone(pos, (33, 35), 50.0), rho)
+    s = 2.0 ** k
+    b = tsp_forward(Grid(e.r * s, e.theta, e.phi), Geometry.cone(pos * s, (33, 35), 50.0), rho)
+    assert float(a.max()) > 0.0 and torch.equal(b / s, a)
