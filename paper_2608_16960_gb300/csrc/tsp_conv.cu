@@ -860,28 +860,41 @@ __global__ void __launch_bounds__(256, 1) wgrad32_tc_kernel(const __grid_constan
     __syncwarp();
   } else if (warp >= 4) {  // ---- epilogue: the CTA's partial dW ----
     // meanwhile: the column sums of Gz (the bias gradient) from the unrotated
-    // copy; a thread adds its eight channels of every 32nd azimuth, in order
+    // copy; a thread adds its eight channels of every 32nd azimuth, in order:
+    // a row's (at most six) plainly, the rows with the remainder of each
+    // addition kept (a plain chain over all of a CTA's rows, 485 values at
+    // batch 8 of 64 x 48 x 96, is off by its length)
     const int c8 = tid & 3, u0 = (tid - 128) >> 2;
-    float cs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    float cs[8], rem[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) cs[i] = rem[i] = 0.0f;
     for (int gi = 0; gi < int(row1 - row0); ++gi) {
       const int gs = gi % NG;
       if (!__all_sync(0xffffffffu, tc_wait(&gfull[gs], uint32_t(gi / NG) & 1u, &s_abort, budget))) break;
       unsigned char* const g = gbase + size_t(gs) * SLOT + ROW;
+      float rs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       for (int u = u0; u < Na; u += 32) {
         const uint4 v = *row_chunk(g, u, c8);
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[i]));
-          cs[2 * i] += f.x;
-          cs[2 * i + 1] += f.y;
+          rs[2 * i] += f.x;
+          rs[2 * i + 1] += f.y;
         }
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float t = cs[i] + rs[i], z = t - cs[i];
+        rem[i] += (cs[i] - (t - z)) + (rs[i] - z);
+        cs[i] = t;
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&gempty[gs]);
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i) {  // the 8 threads of a channel group in a warp, then the 4 warps in order
+      if (rem[i] == rem[i]) cs[i] += rem[i];  // (an infinite sum has no remainder)
       cs[i] += __shfl_xor_sync(0xffffffffu, cs[i], 4);
       cs[i] += __shfl_xor_sync(0xffffffffu, cs[i], 8);
       cs[i] += __shfl_xor_sync(0xffffffffu, cs[i], 16);

@@ -377,3 +377,32 @@ def test_units_of_length(k):
     s = 2.0 ** k
     b = tsp_forward(Grid(e.r * s, e.theta, e.phi), Geometry.cone(pos * s, (33, 35), 50.0), rho)
     assert float(a.max()) > 0.0 and torch.equal(b / s, a)
+
+
+def test_bias_gradients_of_long_rows_of_partial_sums():
+    """A large value at the start of every multiprocessor's share of the rows
+    and then ones that a running float32 sum of it rounds, each by the same
+    2^-7: 430 of them a thread would lose 6e-6 of the sum. Every gradient value
+    is exact in bfloat16 (pass-through layers, a power-of-two mean), so what
+    remains is the sums' rounding: at most 2 plain additions a row, one
+    remainder, 3 shuffles, 4 warps, 8 rows of partial sums and the last
+    addition, 20 ulps in all."""
+    from oracle import net as onet
+    from paper_2608_16960_gb300.model import WarmStartNet
+    batch, shape = 8, (64, 64, 64)
+    net = WarmStartNet(shape, batch)
+    params = [(np.zeros_like(w), np.full_like(b, 2.0 ** -10)) for w, b in onet.init_params(3)]
+    params[5][0][13, 0, :] = (-1.0) ** np.arange(32)
+    params[5][1][:] = 0.0
+    net.set_params(np.concatenate([np.concatenate([w.ravel(), b.ravel()]) for w, b in params]))
+    rows, n = batch * shape[0] * shape[1], batch * int(np.prod(shape))
+    g = np.full((rows, shape[2]), 1.0 + 2.0 ** -7)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    g[rows * np.arange(sms) // sms] = 2.0 ** 18
+    t = torch.tensor((-g * (n / 2)).astype(np.float32).reshape((batch,) + shape), device="cuda")
+    net.loss_grad(torch.zeros_like(t), t)
+    got = net.get_grads()
+    for layer in (1, 2, 3, 4):
+        off, sh = net.layout()[2 * layer + 1]
+        ref = g.sum() * (-1.0) ** np.arange(32)
+        assert (np.abs(got[off:off + 32] - ref) <= 20 * 2.0 ** -24 * np.abs(ref)).all(), layer
