@@ -180,7 +180,6 @@ struct AttenBwdOp {
   float* __restrict__ g_rho;
   float* __restrict__ g_sigma;  // may be null
   float* __restrict__ g_tau1;   // may be null
-  float *sum_a, *sum_b;         // if not null, the voxels' sums of ga and gb instead of the gradients
   RunJoin run;
   float tau2, pre, Y, w;
   __device__ __forceinline__ void step(int v, float dl, float r, float s, float t1) {
@@ -189,14 +188,9 @@ struct AttenBwdOp {
     pre = fmaf(__fmul_rn(r, expf(-__fadd_rn(t1, tau2))), dl, pre);
     const float ga = __fmul_rn(__fmul_rn(w, expf(-tau2)), dl);  // d/d(e^{-tau_1} rho)
     const float gb = -__fmul_rn(__fmul_rn(w, dl), S);           // d/d(sigma rho)
+    const float e1 = expf(-t1);
     LaneSum<MODE> lanes;
     lanes.set(v);
-    if (sum_a) {
-      scatter_add(lanes, sum_a + v, ga);
-      scatter_add(lanes, sum_b + v, gb);
-      return;
-    }
-    const float e1 = expf(-t1);
     scatter_add(lanes, g_rho + v, fmaf(ga, e1, __fmul_rn(gb, s)));
     if (g_sigma) scatter_add(lanes, g_sigma + v, __fmul_rn(gb, r));
     if (g_tau1) scatter_add(lanes, g_tau1 + v, -__fmul_rn(__fmul_rn(ga, r), e1));
@@ -224,31 +218,14 @@ struct AttenBwdOp {
   __device__ __forceinline__ void end(int64_t) { flush(); }
 };
 
-// The factors of a segment's gradients that belong to its voxel are the same
-// for every ray, so a backward pass that overwrites its outputs scatters the
-// sums without them, held in the outputs themselves, and multiplies once per
-// voxel: two atomics and two exponentials a segment instead of three each, one
-// and no gathers in the optical depth's. A sum of zero (a voxel that no ray
-// crosses) gives zero whatever its density. On GB300, 8 views of 256^2 on 60 x
-// 45 x 90: 575 -> 508 us, and the adjoint of tau_1 298 -> 156.
-__global__ void atten_grads_kernel(const float* __restrict__ rho, const float* __restrict__ sigma,
-                                   const float* __restrict__ tau1, float* sum_a, float* sum_b, float* g_rho,
-                                   float* g_sigma, float* g_tau1, int64_t n) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
-    const float a = sum_a[i], b = sum_b[i], r = rho[i];
-    float gr = 0.0f, gs = 0.0f, gt = 0.0f;
-    if (a != 0.0f || b != 0.0f) {
-      const float e1 = expf(-tau1[i]);
-      gr = fmaf(a, e1, __fmul_rn(b, sigma[i]));
-      gs = __fmul_rn(b, r);
-      gt = -__fmul_rn(__fmul_rn(a, r), e1);
-    }
-    g_rho[i] = gr;
-    if (g_sigma) g_sigma[i] = gs;
-    if (g_tau1) g_tau1[i] = gt;
-  }
-}
-
+// The factor of a segment's gradient that belongs to its voxel is the same for
+// every ray, so an adjoint of the optical depth that overwrites its outputs
+// scatters the sums without it, held in g_rho, and multiplies once per voxel:
+// one atomic and no gathers a segment. A sum of zero (a voxel that no ray
+// crosses) gives zero whatever its density. On GB300, the solar rays of 60 x 45
+// x 90: 298 -> 156 us. (The backward pass along the sight lines by two such
+// sums takes 508 us instead of 575 for 8 views of 256^2, but g_rho's two terms
+// cancel in part, and summed apart they were 3% further from 64 bits.)
 // g_rho (the scattered sum) -> sigma g_rho, g_sigma = rho g_rho
 __global__ void product_grads_kernel(const float* __restrict__ rho, const float* __restrict__ sigma, float* g_rho,
                                      float* g_sigma, int64_t n) {
@@ -297,7 +274,7 @@ void launch_product_scatter(tsp_grid grid, tsp_geom sun, const tsp_launch& l, co
 template <int MODE>
 void launch_atten_bwd(tsp_grid grid, tsp_geom geom, const tsp_launch& l, const float* rho, const float* sigma,
                       const float* tau1, const float* y, const float* gy, float* g_rho, float* g_sigma,
-                      float* g_tau1, float* sum_a, float* sum_b, int b, cudaStream_t cs) {
+                      float* g_tau1, int b, cudaStream_t cs) {
   const int64_t V = grid->voxels(), n = geom->n_rays;
   AttenBwdOp<MODE> op;
   op.rho = rho + b * V;
@@ -308,8 +285,6 @@ void launch_atten_bwd(tsp_grid grid, tsp_geom geom, const tsp_launch& l, const f
   op.g_rho = g_rho + b * V;
   op.g_sigma = g_sigma ? g_sigma + b * V : nullptr;
   op.g_tau1 = g_tau1 ? g_tau1 + b * V : nullptr;
-  op.sum_a = sum_a ? sum_a + b * V : nullptr;
-  op.sum_b = sum_b ? sum_b + b * V : nullptr;
   launch_trace(grid, geom, l, op, cs);
 }
 
@@ -431,22 +406,15 @@ extern "C" tsp_status tsp_atten_backward(tsp_grid grid, tsp_geom geom, const flo
     if (g_sigma) TSP_CUDA(cudaMemsetAsync(g_sigma, 0, bytes, cs));
     if (g_tau1) TSP_CUDA(cudaMemsetAsync(g_tau1, 0, bytes, cs));
   }
-  // the sums of ga and gb in two of the outputs, where they are overwritten
-  float *sum_a = nullptr, *sum_b = nullptr;
-  if (!accumulate && g_sigma) sum_a = g_rho, sum_b = g_sigma;
-  else if (!accumulate && g_tau1) sum_a = g_tau1, sum_b = g_rho;
   const Combine mode = combine_of(grid, geom, l, values);
   for (int b = 0; b < batch; ++b) {
     if (mode == COMBINE_RUNS)
-      launch_atten_bwd<COMBINE_RUNS>(grid, geom, l, rho, sigma, tau1, y, gy, g_rho, g_sigma, g_tau1, sum_a, sum_b, b, cs);
+      launch_atten_bwd<COMBINE_RUNS>(grid, geom, l, rho, sigma, tau1, y, gy, g_rho, g_sigma, g_tau1, b, cs);
     else if (mode == COMBINE_PAIRS)
-      launch_atten_bwd<COMBINE_PAIRS>(grid, geom, l, rho, sigma, tau1, y, gy, g_rho, g_sigma, g_tau1, sum_a, sum_b, b, cs);
+      launch_atten_bwd<COMBINE_PAIRS>(grid, geom, l, rho, sigma, tau1, y, gy, g_rho, g_sigma, g_tau1, b, cs);
     else
-      launch_atten_bwd<COMBINE_NONE>(grid, geom, l, rho, sigma, tau1, y, gy, g_rho, g_sigma, g_tau1, sum_a, sum_b, b, cs);
+      launch_atten_bwd<COMBINE_NONE>(grid, geom, l, rho, sigma, tau1, y, gy, g_rho, g_sigma, g_tau1, b, cs);
   }
-  if (sum_a)
-    atten_grads_kernel<<<voxel_blocks(V * batch), 256, 0, cs>>>(rho, sigma, tau1, sum_a, sum_b, g_rho, g_sigma, g_tau1,
-                                                                V * batch);
   TSP_CUDA(cudaGetLastError());
   return TSP_OK;
 }

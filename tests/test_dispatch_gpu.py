@@ -406,3 +406,22 @@ def test_bias_gradients_of_long_rows_of_partial_sums():
         off, sh = net.layout()[2 * layer + 1]
         ref = g.sum() * (-1.0) ** np.arange(32)
         assert (np.abs(got[off:off + 32] - ref) <= 20 * 2.0 ** -24 * np.abs(ref)).all(), layer
+
+
+def test_attenuated_density_gradient_of_cancelling_terms():
+    """One voxel, 4096 times the same ray: each ray's two terms of the density
+    gradient cancel to a thousandth, so the sum of their small remainders has
+    to be that of one ray times 4096, within the rounding of 4096 additions
+    (2^-24 of the sum each), not that of either term's."""
+    from paper_2608_16960_gb300.projector import atten_backward, atten_forward
+    grid = Grid(np.array([0.0, 2.0]), np.array([0.0, np.pi]), np.array([0.0, 2.0 * np.pi]))
+    chord, full = 2.0 * np.sqrt(4.0 - 0.3 ** 2 - 0.4 ** 2), lambda v: torch.full((1, 1, 1), v, device="cuda")
+    rho, sigma, tau1 = full(0.5), full(1.001 / (0.5 * chord)), full(0.2)
+    got = []
+    for n in (1, 4096):
+        x, d = (torch.tensor(v, device="cuda").reshape(3, 1).repeat(1, n) for v in ([-5.0, 0.3, 0.4], [1.0, 0.0, 0.0]))
+        geom = Geometry.rays(x, d)
+        y = atten_forward(grid, geom, rho, sigma, tau1)
+        got.append(float(atten_backward(grid, geom, rho, sigma, tau1, y, torch.ones(n, device="cuda"))[0]))
+    assert 0.0 < abs(got[0]) < 0.01
+    assert abs(got[1] - 4096 * got[0]) <= 4096 * 2.0 ** -24 * abs(4096 * got[0]), got
