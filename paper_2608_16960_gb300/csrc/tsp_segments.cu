@@ -211,13 +211,15 @@ tsp_status exclusive_scan(const int* in, int64_t n, int64_t* out, int64_t* sums,
   return TSP_OK;
 }
 
-// Row offsets of the sorted entries: off[v] = entries with a key below v.
-__global__ void key_offsets_kernel(const uint32_t* __restrict__ keys, int64_t S, int64_t n_rows,
-                                   int64_t* __restrict__ off) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i <= S; i += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t lo = i == 0 ? -1 : int64_t(min(keys[i - 1], uint32_t(n_rows - 1)));
-    const int64_t hi = i == S ? n_rows : int64_t(min(keys[i], uint32_t(n_rows - 1)));
-    for (int64_t v = lo + 1; v <= hi; ++v) off[v] = i;
+// Entries per key of the sorted keys (cnt zeroed before): a key's first entry
+// subtracts its index, its last adds one more than its own.
+__global__ void key_counts_kernel(const uint32_t* __restrict__ keys, int64_t S, uint32_t key_max,
+                                  unsigned* __restrict__ cnt) {
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < S; i += int64_t(gridDim.x) * blockDim.x) {
+    const uint32_t k = keys[i];
+    const uint32_t at = min(k, key_max);  // the clamp only guards memory
+    if (i == 0 || keys[i - 1] != k) atomicAdd(cnt + at, 0u - unsigned(i));
+    if (i == S - 1 || keys[i + 1] != k) atomicAdd(cnt + at, unsigned(i) + 1u);
   }
 }
 
@@ -835,7 +837,7 @@ static tsp_status build_lists(tsp_grid grid, tsp_geom geom, int transpose, Block
   const int64_t n_rt = (S + RT - 1) / RT;
   uint32_t *xi = nullptr, *ka = nullptr, *kb = nullptr, *rb = nullptr;
   float *xl = nullptr, *lb = nullptr;
-  int* rhist = nullptr;
+  int *rhist = nullptr, *vcount = nullptr;
   int64_t *rbase = nullptr, *rsums = nullptr;
   entries.add(&f.off, n_rays + 1);
   entries.add(&f.idx, S);
@@ -854,7 +856,8 @@ static tsp_status build_lists(tsp_grid grid, tsp_geom geom, int transpose, Block
     }
     second.add(&rhist, RD * n_rt);
     second.add(&rbase, RD * n_rt + 1);
-    second.add(&rsums, scan_words(RD * n_rt));
+    second.add(&vcount, V);
+    second.add(&rsums, scan_words(std::max(RD * n_rt, V)));
   }
   SEG_TRY(entries.allocate(lists));
   SEG_TRY(second.allocate(scratch, 1));
@@ -894,7 +897,11 @@ static tsp_status build_lists(tsp_grid grid, tsp_geom geom, int transpose, Block
         il = ol;
       }
     }
-    key_offsets_kernel<<<152 * 16, 256, 0, cs>>>(ka, S, V, t.off);
+    SEG_TRY(cudaMemsetAsync(vcount, 0, sizeof(int) * size_t(V), cs));
+    if (S > 0)
+      key_counts_kernel<<<152 * 16, 256, 0, cs>>>(ka, S, uint32_t(V - 1), reinterpret_cast<unsigned*>(vcount));
+    st = exclusive_scan(vcount, V, t.off, rsums, cs);
+    if (st != TSP_OK) return bail(st);
     SEG_TRY(cudaGetLastError());
     s->has_adj = true;
   }

@@ -425,3 +425,26 @@ def test_attenuated_density_gradient_of_cancelling_terms():
         got.append(float(atten_backward(grid, geom, rho, sigma, tau1, y, torch.ones(n, device="cuda"))[0]))
     assert 0.0 < abs(got[0]) < 0.01
     assert abs(got[1] - 4096 * got[0]) <= 4096 * 2.0 ** -24 * abs(4096 * got[0]), got
+
+
+@pytest.mark.parametrize("fov,empty", [(0.02, False), (8.0, True)])
+def test_lists_of_a_large_grid_that_few_rays_meet(fov, empty):
+    """Voxel offsets of 64 M voxels of which next to none have entries: right,
+    and written by all of the GPU (under 20 ms; one thread over the gap takes
+    hundreds)."""
+    import time
+    from paper_2608_16960_gb300.projector import Segments
+    grid, _ = _grid((250, 256, 1000))
+    pos = synth.circular_orbit(1, 60.0, incline_deg=20.0, phase=0.3)
+    geom = Geometry.cone(pos, (8, 8), fov, look_at=2.0 * pos if empty else None)
+    Segments(grid, geom)
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    s = Segments(grid, geom)
+    torch.cuda.synchronize()
+    t = time.perf_counter() - t0
+    off, vox, _ = s.export()
+    assert (off[-1] == 0) == empty
+    voff = s.export_transposed()[0]
+    assert np.array_equal(np.diff(voff), np.bincount(vox, minlength=grid.voxels))
+    assert t < 0.02, t
