@@ -168,8 +168,13 @@ tsp_status tsp_count_segments(tsp_grid grid, tsp_geom geom, int* counts, void* s
  * adjoint is a per-voxel gather instead of a per-segment scatter. The
  * transpose is a stable radix sort by voxel (8 key bits per pass), so each
  * voxel's list is in ray-major order and the lists, and every result computed
- * from them, are the same on every build; it takes 16 to 24 bytes per segment of
- * temporary device memory during the build.
+ * from them, are the same on every build.
+ *
+ * Temporary device memory of a build: 16 bytes per ray, and without the
+ * transpose 8 bytes per segment, 512 MB at most (less where the device has
+ * less; larger lists are filled in pieces, a walk of the rays each). With it 24
+ * bytes per ray, 4 per voxel and 18 per segment; where those do not fit, 6 to 14
+ * per segment (by the number of key bits) and one more walk.
  *
  * The segments are those tsp_forward walks: lists and on-the-fly traversal
  * give the same F up to float32 rounding order. Forward and adjoint read the
@@ -255,6 +260,13 @@ tsp_status tsp_segments_sirt_weights(tsp_segments s, float* R, float* C, void* s
  */
 tsp_status tsp_debug_fail_allocation(int64_t after);
 tsp_status tsp_debug_allocation_count(int64_t* count);
+/*
+ * tsp_debug_segments_memory - test hook: in stored-list builds arrays that
+ * together exceed block_most bytes get an allocation each (default 512 MB), and
+ * scratch per segment above scratch_most bytes counts as not available (default:
+ * no limit). Negative values restore the defaults. Process-wide.
+ */
+tsp_status tsp_debug_segments_memory(int64_t block_most, int64_t scratch_most);
 tsp_status tsp_segments_sirt(tsp_segments s, const float* y, float* x, int n_iter, int flags,
                              void* workspace, size_t workspace_bytes, void* stream);
 void tsp_segments_destroy(tsp_segments s);

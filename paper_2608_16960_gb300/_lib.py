@@ -64,6 +64,7 @@ SIGNATURES = {
     "tsp_segments_export_transposed": (_I, [_P, _P, _P, _P]),
     "tsp_segments_sirt_weights": (_I, [_P, _P, _P, _P]),
     "tsp_debug_fail_allocation": (_I, [_I64]),
+    "tsp_debug_segments_memory": (_I, [_I64, _I64]),
     "tsp_debug_allocation_count": (_I, [_I64P]),
     "tsp_debug_tc_stall": (_I, [_I64]),
     "tsp_segments_forward": (_I, [_P, _P, _P, _I, _P]),

@@ -6,6 +6,9 @@
 // these lists stream 8 bytes per segment: the lists are read once, coalesced,
 // and multiply an input gathered from L2 (the volume, or the detector values),
 // summed per output row in registers.
+#include <atomic>
+#include <limits>
+
 #include "tsp_kernels.cuh"
 
 // One direction of the lists: rows (rays or voxels) with their entries
@@ -28,6 +31,13 @@ struct RowOrder {
     const int h = H - 4 * int(band) < 4 ? H - 4 * int(band) : 4;
     const int64_t col = in_band / h, row = 4 * band + (in_band - col * h);
     return (view * H + row) * W + col;
+  }
+  __host__ __device__ int64_t row(int64_t r) const {  // ray's inverse
+    if (W == 0) return r;
+    const int64_t view = r / (int64_t(H) * W);
+    const int in_view = int(r - view * (int64_t(H) * W)), i = in_view / W, col = in_view - i * W, band = i / 4;
+    const int h = H - 4 * band < 4 ? H - 4 * band : 4;
+    return view * (int64_t(H) * W) + 4 * int64_t(band) * W + int64_t(col) * h + (i - 4 * band);
   }
 };
 
@@ -68,9 +78,15 @@ struct CountOnlyOp {
 // guards memory should that ever fail, and flags the error word.
 // Four entries leave at a time (16 bytes of columns, 16 of lengths), the first
 // and last of a row singly: an entry by itself is two 4-byte writes to lines of
-// its own (11 M segments of 0.3 M rays, 206 -> 143 us).
+// its own (11 M segments of 0.3 M rays, 206 -> 143 us). The entries go ray after
+// ray (off: the rays' offsets), or (ROWS) those of the rows p0 .. p1 - 1 row
+// after row from word 0 on (off: the rows' offsets); rays of other rows leave
+// at once.
+template <bool ROWS>
 struct FillOp {
   const int64_t* __restrict__ off;
+  RowOrder order;
+  int64_t p0, p1;
   uint32_t* __restrict__ vox;
   float* __restrict__ len;
   int64_t pos, lim, out;  // entries seen, row end, entries written
@@ -79,8 +95,10 @@ struct FillOp {
   bool bad;
   __device__ __forceinline__ bool begin(int64_t ray) {
     bad = false;
-    pos = out = off[ray];
-    lim = off[ray + 1];
+    const int64_t i = ROWS ? order.row(ray) : ray, base = ROWS ? off[p0] : 0;
+    if (ROWS && (i < p0 || i >= p1)) return false;
+    pos = out = off[i] - base;
+    lim = off[i + 1] - base;
     v0 = v1 = v2 = 0u;
     l0 = l1 = l2 = 0.0f;
     return true;
@@ -223,6 +241,13 @@ __global__ void key_counts_kernel(const uint32_t* __restrict__ keys, int64_t S, 
   }
 }
 
+// Offsets of the keys below 2^RB after one pass: where each digit begins.
+__global__ void digit_offsets_kernel(const int64_t* __restrict__ base, int64_t n_tiles, int64_t n_rows,
+                                     int64_t* __restrict__ off) {
+  const int64_t v = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (v <= n_rows) off[v] = base[v * n_tiles];
+}
+
 // ---- voxel-major transpose: stable LSD radix sort of the entries by voxel ----
 // Keys are the voxel ids of the ray-major entries, carried with their ray id
 // and length, RB bits of the key per pass. A pass counts each tile's digits,
@@ -315,7 +340,7 @@ __global__ void __launch_bounds__(RW * 32) radix_scatter_kernel(
     const uint32_t kk = sk[j];
     const uint32_t d = (kk >> shift) & (RD - 1);
     const int64_t g = base[int64_t(d) * n_tiles + t] + (j - start[d]);
-    keys_out[g] = kk;
+    if (keys_out) keys_out[g] = kk;
     rays_out[g] = sr[j];
     lens_out[g] = sl[j];
   }
@@ -337,18 +362,19 @@ __global__ void order_counts_kernel(const int* __restrict__ counts, int64_t n_ro
   if (row < n_rows) out[row] = counts[order.ray(row)];
 }
 
-// Entries ray after ray (offsets off_in) into the interleaved order: a warp per
-// slice, a row per lane.
-__global__ void __launch_bounds__(256) interleave_kernel(const int64_t* __restrict__ off, int64_t n_rows,
+// Entries into the interleaved order, a warp per slice, a row per lane: from
+// ray after ray (their offsets off_in), or, with off_in NULL, the rows p0 ..
+// n_rows - 1 row after row from word 0 on (p0 a multiple of 32).
+__global__ void __launch_bounds__(256) interleave_kernel(const int64_t* __restrict__ off, int64_t p0, int64_t n_rows,
                                                          RowOrder order, const int64_t* __restrict__ off_in,
                                                          const uint32_t* __restrict__ idx_in,
                                                          const float* __restrict__ len_in,
                                                          uint32_t* __restrict__ idx, float* __restrict__ len) {
-  const int64_t row = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t row = p0 + int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   const unsigned below = (1u << (threadIdx.x & 31)) - 1u;
   const int64_t o0 = off[min(row, n_rows)], o1 = off[min(row + 1, n_rows)];
   const int n = int(o1 - o0), most = __reduce_max_sync(0xffffffffu, n);
-  const int64_t from = row < n_rows ? off_in[order.ray(row)] : 0;
+  const int64_t from = off_in == nullptr ? o0 - off[p0] : (row < n_rows ? off_in[order.ray(row)] : 0);
   int64_t q = __shfl_sync(0xffffffffu, o0, 0);
 #pragma unroll 4
   for (int k = 0; k < most; ++k) {
@@ -679,14 +705,18 @@ struct Blocks {
   }
 };
 
+// Limits that tsp_debug_segments_memory changes: the largest block of several
+// arrays, and the most scratch per segment that a build may take.
+constexpr int64_t BLOCK_MOST = int64_t(512) << 20;
+std::atomic<int64_t> g_block_most{BLOCK_MOST}, g_scratch_most{std::numeric_limits<int64_t>::max()};
+
 // Several arrays in one device allocation, 256-byte aligned each (in the spare
 // one if it is large enough), as long as they are small: an allocation and its
 // release take some 60 us however few bytes they are of. Together above
-// CARVE_MOST bytes each gets its own: the driver clears a large block that was
+// BLOCK_MOST bytes each gets its own: the driver clears a large block that was
 // freed behind the kernels that follow (a first pass over 2.5 GB of lists took
 // 530 us instead of 320 after a build with its scratch in one block). Every
 // array passes the allocation hook, so a test can fail any of them.
-constexpr size_t CARVE_MOST = size_t(512) << 20;
 struct Carve {
   std::vector<std::pair<void**, size_t>> parts;
   template <class T>
@@ -698,15 +728,23 @@ struct Carve {
     for (const auto& p : parts) b += p.second;
     return b;
   }
-  cudaError_t allocate(Blocks& blocks, int spare = -1) const {  // spare: the block to use or to become
+  // spare: the block to use or to become. On failure nothing is held that was not before; *injected: by the test hook.
+  cudaError_t allocate(Blocks& blocks, int spare = -1, bool* injected = nullptr) const {
     for (size_t i = 0; i < parts.size(); ++i) {
       const cudaError_t e = dev_malloc_hook();
-      if (e != cudaSuccess) return e;
+      if (e != cudaSuccess) {
+        if (injected) *injected = true;
+        return e;
+      }
     }
-    if (bytes() > CARVE_MOST) {
+    if (int64_t(bytes()) > g_block_most.load()) {
+      const size_t before = blocks.held.size();
       for (const auto& p : parts) {
         const cudaError_t e = cudaMalloc(p.first, p.second);
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess) {
+          for (; blocks.held.size() > before; blocks.held.pop_back()) cudaFree(blocks.held.back());
+          return e;
+        }
         blocks.held.push_back(*p.first);
       }
       return cudaSuccess;
@@ -750,6 +788,70 @@ extern "C" void tsp_segments_destroy(tsp_segments s) {
   if (!s) return;
   for (void* p : s->held) cudaFree(p);
   delete s;
+}
+
+// The rows' entries into the interleaved order, from the walk in pieces of whole
+// slices through a staging buffer, so that lists of any size take a bounded
+// scratch: each piece is one more walk in which the rays of other pieces leave
+// at once (200 M segments of 3 M rays in 256 MB: 7 pieces).
+constexpr int64_t STAGE_MOST = int64_t(512) << 20;
+static tsp_status fill_rows(tsp_grid grid, tsp_geom geom, const tsp_launch& l, SegList& f, RowOrder order,
+                            cudaStream_t cs) {
+  if (f.S == 0) return TSP_OK;
+  const int64_t n_slices = (f.n_rows + 31) / 32;
+  std::vector<int64_t> first;  // offsets of the slices, once one piece is not enough
+  int64_t widest = f.S;
+  auto slices = [&]() -> tsp_status {
+    first.assign(size_t(n_slices + 1), f.S);
+    TSP_CUDA(cudaMemcpy2DAsync(first.data(), sizeof(int64_t), f.off, 32 * sizeof(int64_t), sizeof(int64_t),
+                               size_t(n_slices), cudaMemcpyDeviceToHost, cs));
+    TSP_CUDA(cudaStreamSynchronize(cs));
+    widest = 0;
+    for (int64_t k = 0; k < n_slices; ++k) widest = std::max(widest, first[size_t(k + 1)] - first[size_t(k)]);
+    return TSP_OK;
+  };
+  int64_t most = std::min(f.S, std::min(g_scratch_most.load(), STAGE_MOST) / 8);  // entries
+  if (most < f.S) {
+    const tsp_status st = slices();
+    if (st != TSP_OK) return st;
+    most = std::max(most, widest);
+  }
+  uint32_t* xi = nullptr;
+  if (dev_malloc_hook() != cudaSuccess) return fail(TSP_ENOMEM, "tsp_segments_build: out of device memory (staging)");
+  for (;;) {  // (the lengths after the columns, on a multiple of four entries)
+    const cudaError_t e = cudaMalloc(&xi, size_t(8 * ((most + 3) & ~int64_t(3))));
+    if (e == cudaSuccess) break;
+    cudaGetLastError();  // not sticky: clear it
+    if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "tsp_segments_build: staging");
+    if (first.empty()) {
+      const tsp_status st = slices();
+      if (st != TSP_OK) return st;
+    }
+    if (most / 2 < std::max(widest, int64_t(1) << 17))
+      return fail(TSP_ENOMEM, "tsp_segments_build: out of device memory (staging)");
+    most /= 2;
+  }
+  float* xl = reinterpret_cast<float*>(xi + ((most + 3) & ~int64_t(3)));
+  for (int64_t s0 = 0, s1; s0 < n_slices; s0 = s1) {
+    s1 = n_slices;
+    if (!first.empty())
+      for (s1 = s0 + 1; s1 < n_slices && first[size_t(s1 + 1)] - first[size_t(s0)] <= most;) ++s1;
+    FillOp<true> op;
+    op.off = f.off;
+    op.order = order;
+    op.p0 = 32 * s0;
+    op.p1 = std::min(32 * s1, f.n_rows);
+    op.vox = xi;
+    op.len = xl;
+    launch_trace(grid, geom, l, op, cs);
+    interleave_kernel<<<unsigned((op.p1 - op.p0 + 255) / 256), 256, 0, cs>>>(f.off, op.p0, op.p1, order, nullptr, xi,
+                                                                            xl, f.idx, f.len);
+  }
+  cudaError_t e = cudaGetLastError();
+  const cudaError_t done = cudaStreamSynchronize(cs);
+  cudaFree(xi);
+  if (e == cudaSuccess) e = done;
+  return e == cudaSuccess ? TSP_OK : cuda_fail(e, "tsp_segments_build: filling the lists");
 }
 
 // One allocation for the lists and two for the build's scratch: with one per
@@ -800,92 +902,113 @@ static tsp_status build_lists(tsp_grid grid, tsp_geom geom, int transpose, Block
   SegList &f = s->fwd, &t = s->adj;
   f.n_rows = t.n_cols = n_rays;
   f.n_cols = t.n_rows = V;
-  Carve entries, first, second;
+  Carve entries, first;
   int *counts = nullptr, *ordered = nullptr;
   int64_t *ray_off = nullptr, *row_off = nullptr, *sums = nullptr;
   first.add(&counts, n_rays);
   first.add(&ordered, n_rays);
-  first.add(&ray_off, n_rays + 1);
   first.add(&row_off, n_rays + 1);
   first.add(&sums, scan_words(n_rays));
+  if (transpose) first.add(&ray_off, n_rays + 1);
   SEG_TRY(first.allocate(scratch, 0));
   const tsp_launch l = preferred_launch(grid, geom, false);
   CountOnlyOp cop;
   cop.counts = counts;
   launch_trace(grid, geom, l, cop, cs);
-  st = exclusive_scan(counts, n_rays, ray_off, sums, cs);
-  if (st != TSP_OK) return bail(st);
   const unsigned row_blocks = unsigned((n_rays + 255) / 256);
   order_counts_kernel<<<row_blocks, 256, 0, cs>>>(counts, n_rays, s->order, ordered);
   st = exclusive_scan(ordered, n_rays, row_off, sums, cs);
+  if (st == TSP_OK && transpose) st = exclusive_scan(counts, n_rays, ray_off, sums, cs);
   if (st != TSP_OK) return bail(st);
-  SEG_TRY(cudaMemcpyAsync(&s->n_segs, ray_off + n_rays, sizeof(int64_t), cudaMemcpyDeviceToHost, cs));
+  SEG_TRY(cudaMemcpyAsync(&s->n_segs, row_off + n_rays, sizeof(int64_t), cudaMemcpyDeviceToHost, cs));
   SEG_TRY(cudaStreamSynchronize(cs));
   const int64_t S = s->n_segs;
   if (S >= (int64_t(1) << 32)) return bail(fail(TSP_ENOTSUP, "tsp_segments_build: 2^32 or more segments"));
   f.S = t.S = S;
-  // Radix sort by voxel: `passes` stable passes between the buffers A = (ka,
-  // t.idx, t.len) and B = (kb, rb, lb) of (key, ray, length), so that the last
-  // one reads B and writes A; its keys give the row offsets. The first reads the row-major
-  // entries X and their ray ids, which start in the ray array that it does not
-  // write. With three passes (up to 2^24 voxels) it writes A, and B's keys and
-  // lengths may take X's place.
-  int bits = 1;
-  while (bits < 32 && (uint64_t(V - 1) >> bits) != 0) ++bits;
-  const int passes = (bits + RB - 1) / RB;
-  const bool first_to_a = (passes - 1) % 2 == 0;
-  const int64_t n_rt = (S + RT - 1) / RT;
-  uint32_t *xi = nullptr, *ka = nullptr, *kb = nullptr, *rb = nullptr;
-  float *xl = nullptr, *lb = nullptr;
-  int *rhist = nullptr, *vcount = nullptr;
-  int64_t *rbase = nullptr, *rsums = nullptr;
   entries.add(&f.off, n_rays + 1);
   entries.add(&f.idx, S);
   entries.add(&f.len, S);
-  second.add(&xi, S);
-  second.add(&xl, S);
   if (transpose) {
     entries.add(&t.off, V + 1);
     entries.add(&t.idx, S);
     entries.add(&t.len, S);
-    second.add(&rb, S);
-    second.add(&ka, S);
-    if (passes > 1 && !first_to_a) {
-      second.add(&kb, S);
-      second.add(&lb, S);
-    }
-    second.add(&rhist, RD * n_rt);
-    second.add(&rbase, RD * n_rt + 1);
-    second.add(&vcount, V);
-    second.add(&rsums, scan_words(std::max(RD * n_rt, V)));
   }
   SEG_TRY(entries.allocate(lists));
-  SEG_TRY(second.allocate(scratch, 1));
   SEG_TRY(cudaMemcpyAsync(f.off, row_off, sizeof(int64_t) * size_t(n_rays + 1), cudaMemcpyDeviceToDevice, cs));
-  if (first_to_a) {
-    kb = xi;
-    lb = xl;
-  }
-  FillOp fop;
-  fop.off = ray_off;
-  fop.vox = xi;
-  fop.len = xl;
-  launch_trace(grid, geom, l, fop, cs);
-  interleave_kernel<<<row_blocks, 256, 0, cs>>>(f.off, n_rays, s->order, ray_off, xi, xl, f.idx, f.len);
-  SEG_TRY(cudaGetLastError());
-  if (transpose) {
+  if (!transpose) {
+    st = fill_rows(grid, geom, l, f, s->order, cs);
+    if (st != TSP_OK) return bail(st);
+  } else {
+    // Radix sort by voxel of the entries ray after ray, X: `passes` stable passes
+    // between the buffers A = (ka, t.idx, t.len) and B = (kb, rb, lb) of (key,
+    // ray, length), so that the last one reads B and writes A; its keys give
+    // the row offsets. The first reads X and its ray ids, which start in the ray
+    // array that it does not write. f holds nothing of its own until the end:
+    // with X in scratch it is B's keys and lengths, and X is interleaved into
+    // it last (16 bytes a segment of scratch, 12 for one pass). Where that does
+    // not fit, X is filled into f and gives up its place to the sort after the
+    // first pass (4, 12, 8, 12 bytes for one to four passes), and f is filled by
+    // one more walk.
+    int bits = 1;
+    while (bits < 32 && (uint64_t(V - 1) >> bits) != 0) ++bits;
+    const int passes = (bits + RB - 1) / RB;
+    const bool first_to_a = (passes - 1) % 2 == 0;
+    const int64_t n_rt = (S + RT - 1) / RT;
+    uint32_t *xi = nullptr, *ka = nullptr, *kb = nullptr, *rb = nullptr;
+    float *xl = nullptr, *lb = nullptr;
+    int *rhist = nullptr, *vcount = nullptr;
+    int64_t *rbase = nullptr, *rsums = nullptr;
+    bool in_place = false;
+    for (;; in_place = true) {
+      Carve second;
+      second.add(&rb, S);
+      if (!in_place) {
+        second.add(&xi, S);
+        second.add(&xl, S);
+        if (passes > 1) second.add(&ka, S);
+      } else if (passes > 1 && first_to_a) {
+        second.add(&ka, S);
+      } else if (passes > 1) {
+        second.add(&kb, S);
+        second.add(&lb, S);
+      }
+      second.add(&rhist, RD * n_rt);
+      second.add(&rbase, RD * n_rt + 1);
+      second.add(&vcount, V);
+      second.add(&rsums, scan_words(std::max(RD * n_rt, V)));
+      bool injected = false;
+      const cudaError_t e = int64_t(second.bytes()) > g_scratch_most.load() ? cudaErrorMemoryAllocation
+                                                                           : second.allocate(scratch, 1, &injected);
+      if (e == cudaSuccess) break;
+      if (e != cudaErrorMemoryAllocation || in_place || injected) SEG_TRY(e);
+      cudaGetLastError();  // not sticky: clear it
+    }
+    if (in_place) {
+      xi = f.idx;
+      xl = f.len;
+    }
+    if (!in_place || first_to_a) {
+      kb = f.idx;
+      lb = f.len;
+    } else {
+      ka = f.idx;
+    }
+    FillOp<false> fop;
+    fop.off = ray_off;
+    fop.vox = xi;
+    fop.len = xl;
+    launch_trace(grid, geom, l, fop, cs);
     if (S > 0) {
       uint32_t* rid = first_to_a ? rb : t.idx;
       ray_ids_kernel<<<unsigned((n_rays * 32 + 255) / 256), 256, 0, cs>>>(ray_off, n_rays, rid);
       const uint32_t *ik = xi, *ir = rid;
       const float* il = xl;
       for (int p = 0; p < passes; ++p) {
-        const bool final_pass = p == passes - 1;
         const int shift = p * RB;
         radix_hist_kernel<<<unsigned(n_rt), RW * 32, 0, cs>>>(ik, S, shift, n_rt, rhist);
         st = exclusive_scan(rhist, RD * n_rt, rbase, rsums, cs);
         if (st != TSP_OK) return bail(st);
-        const bool to_a = final_pass || (passes - 1 - p) % 2 == 0;
+        const bool to_a = (passes - 1 - p) % 2 == 0;
         uint32_t* ok_ = to_a ? ka : kb;
         uint32_t* orr = to_a ? t.idx : rb;
         float* ol = to_a ? t.len : lb;
@@ -897,12 +1020,26 @@ static tsp_status build_lists(tsp_grid grid, tsp_geom geom, int transpose, Block
         il = ol;
       }
     }
-    SEG_TRY(cudaMemsetAsync(vcount, 0, sizeof(int) * size_t(V), cs));
-    if (S > 0)
-      key_counts_kernel<<<152 * 16, 256, 0, cs>>>(ka, S, uint32_t(V - 1), reinterpret_cast<unsigned*>(vcount));
-    st = exclusive_scan(vcount, V, t.off, rsums, cs);
-    if (st != TSP_OK) return bail(st);
+    if (S > 0 && passes == 1) {
+      digit_offsets_kernel<<<unsigned(V / 256 + 1), 256, 0, cs>>>(rbase, n_rt, V, t.off);
+    } else {
+      SEG_TRY(cudaMemsetAsync(vcount, 0, sizeof(int) * size_t(V), cs));
+      if (S > 0)
+        key_counts_kernel<<<152 * 16, 256, 0, cs>>>(ka, S, uint32_t(V - 1), reinterpret_cast<unsigned*>(vcount));
+      st = exclusive_scan(vcount, V, t.off, rsums, cs);
+      if (st != TSP_OK) return bail(st);
+    }
     SEG_TRY(cudaGetLastError());
+    if (!in_place) {
+      interleave_kernel<<<row_blocks, 256, 0, cs>>>(f.off, 0, n_rays, s->order, ray_off, xi, xl, f.idx, f.len);
+      SEG_TRY(cudaGetLastError());
+    } else {
+      SEG_TRY(cudaStreamSynchronize(cs));
+      scratch.release();
+      scratch.release_spares();
+      st = fill_rows(grid, geom, l, f, s->order, cs);
+      if (st != TSP_OK) return bail(st);
+    }
     s->has_adj = true;
   }
   SEG_TRY(cudaStreamSynchronize(cs));
@@ -911,6 +1048,12 @@ static tsp_status build_lists(tsp_grid grid, tsp_geom geom, int transpose, Block
   s->held = lists.held;
   s->bytes = entries.bytes();
   *out = s;
+  return TSP_OK;
+}
+
+extern "C" tsp_status tsp_debug_segments_memory(int64_t block_most, int64_t scratch_most) {
+  g_block_most.store(block_most < 0 ? BLOCK_MOST : block_most);
+  g_scratch_most.store(scratch_most < 0 ? std::numeric_limits<int64_t>::max() : scratch_most);
   return TSP_OK;
 }
 

@@ -448,3 +448,46 @@ def test_lists_of_a_large_grid_that_few_rays_meet(fov, empty):
     voff = s.export_transposed()[0]
     assert np.array_equal(np.diff(voff), np.bincount(vox, minlength=grid.voxels))
     assert t < 0.02, t
+
+
+@pytest.mark.parametrize("shape,n_views,det", [((4, 3, 6), 8, (62, 50)),       # one pass of the sort by voxel
+                                               ((20, 15, 30), 3, (45, 29)),    # two
+                                               ((64, 48, 96), 2, (61, 37)),    # three
+                                               ((260, 256, 256), 1, (23, 21))])  # four
+@pytest.mark.parametrize("kind", ["cone", "rays"])
+def test_lists_built_in_little_memory(shape, n_views, det, kind):
+    """A build that may not take its usual scratch: the sort in the lists' own
+    place and the rows filled in pieces give the same lists, and without the
+    transpose no scratch grows with the segments at all."""
+    from paper_2608_16960_gb300._lib import TspError, load
+    from paper_2608_16960_gb300.projector import Segments
+    grid, _ = _grid(shape)
+    geom = _geometry(kind, n_views, det)
+    L = load()
+    a = Segments(grid, geom)
+    plain, columns = a.export(), a.export_transposed()
+    rho = torch.tensor(synth.uniform_volume(grid.shape, 3, 0.1, 1.0), device="cuda")
+    y = a.forward(rho)
+    S, V = int(plain[0][-1]), grid.voxels
+    tiles = -(-S // 2048)
+    passes = -(-max(1, (V - 1).bit_length()) // 8)
+    need = 4 * (1, 3, 2, 3)[passes - 1] * S + 256 * tiles * 12 + 4 * V + 8 * (max(256 * tiles, V) // 2048) + 4096
+    try:
+        for block in (-1, 0):
+            assert L.tsp_debug_segments_memory(block, need) == 0
+            b = Segments(grid, geom)
+            for u, v in zip(plain + columns, b.export() + b.export_transposed()):
+                assert np.array_equal(u, v)
+            assert torch.equal(b.forward(rho), y)
+            assert L.tsp_debug_segments_memory(block, need - 2 * S) == 0
+            with pytest.raises(TspError) as e:
+                Segments(grid, geom)
+            assert e.value.status == 3  # TSP_ENOMEM
+            for most in (8 * S // 5, 0):
+                assert L.tsp_debug_segments_memory(block, most) == 0
+                c = Segments(grid, geom, transpose=False)
+                for u, v in zip(plain, c.export()):
+                    assert np.array_equal(u, v)
+                assert torch.equal(c.forward(rho), y)
+    finally:
+        L.tsp_debug_segments_memory(-1, -1)
