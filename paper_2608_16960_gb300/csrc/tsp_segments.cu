@@ -716,7 +716,8 @@ std::atomic<int64_t> g_block_most{BLOCK_MOST}, g_scratch_most{std::numeric_limit
 // BLOCK_MOST bytes each gets its own: the driver clears a large block that was
 // freed behind the kernels that follow (a first pass over 2.5 GB of lists took
 // 530 us instead of 320 after a build with its scratch in one block). Every
-// array passes the allocation hook, so a test can fail any of them.
+// array passes the allocation hook: in a block all before its one allocation,
+// else each before its own.
 struct Carve {
   std::vector<std::pair<void**, size_t>> parts;
   template <class T>
@@ -730,17 +731,16 @@ struct Carve {
   }
   // spare: the block to use or to become. On failure nothing is held that was not before; *injected: by the test hook.
   cudaError_t allocate(Blocks& blocks, int spare = -1, bool* injected = nullptr) const {
-    for (size_t i = 0; i < parts.size(); ++i) {
+    auto hook = [&]() {
       const cudaError_t e = dev_malloc_hook();
-      if (e != cudaSuccess) {
-        if (injected) *injected = true;
-        return e;
-      }
-    }
+      if (e != cudaSuccess && injected) *injected = true;
+      return e;
+    };
     if (int64_t(bytes()) > g_block_most.load()) {
       const size_t before = blocks.held.size();
       for (const auto& p : parts) {
-        const cudaError_t e = cudaMalloc(p.first, p.second);
+        cudaError_t e = hook();
+        if (e == cudaSuccess) e = cudaMalloc(p.first, p.second);
         if (e != cudaSuccess) {
           for (; blocks.held.size() > before; blocks.held.pop_back()) cudaFree(blocks.held.back());
           return e;
@@ -748,6 +748,10 @@ struct Carve {
         blocks.held.push_back(*p.first);
       }
       return cudaSuccess;
+    }
+    for (size_t i = 0; i < parts.size(); ++i) {  // one allocation that stands for all of them
+      const cudaError_t e = hook();
+      if (e != cudaSuccess) return e;
     }
     void* block = nullptr;
     if (spare >= 0 && blocks.spare_bytes[spare] >= bytes()) {

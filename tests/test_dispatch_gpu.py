@@ -491,3 +491,52 @@ def test_lists_built_in_little_memory(shape, n_views, det, kind):
                 assert torch.equal(c.forward(rho), y)
     finally:
         L.tsp_debug_segments_memory(-1, -1)
+
+
+@pytest.mark.parametrize("transpose", [True, False])
+@pytest.mark.parametrize("limit", [-1, 1])
+def test_build_out_of_memory_between_single_allocations(transpose, limit):
+    """Lists too large for one block take an allocation an array: whichever of
+    them fails, with the usual scratch or without, the build returns
+    TSP_ENOMEM, frees the ones before it, and the next build succeeds."""
+    import ctypes
+    from paper_2608_16960_gb300._lib import TspError, load
+    from paper_2608_16960_gb300.projector import Segments, tsp_device_status
+    grid, _ = _grid((10, 8, 12))
+    geom = _geometry("cone", 2, (24, 24))
+    L = load()
+    count = ctypes.c_int64()
+
+    def allocations():
+        assert L.tsp_debug_allocation_count(ctypes.byref(count)) == 0
+        return count.value
+
+    ref = Segments(grid, geom, transpose=transpose)
+    S, V = int(ref.export()[0][-1]), grid.voxels
+    tiles = -(-S // 2048)
+    # the transposed build without its scratch of 16 bytes a segment: 12 and what does not grow by segment
+    need = 12 * S + 256 * tiles * 12 + 4 * V + 8 * (max(256 * tiles, V) // 2048) + 4096
+    scratch = -1 if limit < 0 else (need if transpose else 0)
+    rho = torch.tensor(synth.uniform_volume(grid.shape, 3, 0.1, 1.0), device="cuda")
+    y = ref.forward(rho)
+    try:
+        assert L.tsp_debug_segments_memory(0, scratch) == 0
+        n0 = allocations()
+        assert torch.equal(Segments(grid, geom, transpose=transpose).forward(rho), y)
+        n = allocations() - n0
+        assert n >= (18 if transpose else 8)
+        torch.cuda.synchronize()
+        free0 = torch.cuda.mem_get_info()[0]
+        for k in range(n):
+            assert L.tsp_debug_fail_allocation(k) == 0
+            before = allocations()
+            with pytest.raises(TspError) as e:
+                Segments(grid, geom, transpose=transpose)
+            assert e.value.status == 3 and allocations() - before == k + 1  # it stopped at the one that failed
+            assert torch.equal(Segments(grid, geom, transpose=transpose).forward(rho), y)
+    finally:
+        L.tsp_debug_fail_allocation(-1)
+        L.tsp_debug_segments_memory(-1, -1)
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] >= free0 - (64 << 20)
+    assert tsp_device_status() == 0
