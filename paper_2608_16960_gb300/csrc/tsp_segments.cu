@@ -696,12 +696,14 @@ struct Blocks {
     for (void* p : held) cudaFree(p);
     held.clear();
   }
+  void release_spare(int i) {
+    cudaFree(spare[i]);
+    spare[i] = nullptr;
+    spare_bytes[i] = 0;
+  }
   void release_spares() {
-    for (int i = 0; i < 2; ++i) {
-      cudaFree(spare[i]);
-      spare[i] = nullptr;
-      spare_bytes[i] = 0;
-    }
+    release_spare(0);
+    release_spare(1);
   }
 };
 
@@ -737,6 +739,7 @@ struct Carve {
       return e;
     };
     if (int64_t(bytes()) > g_block_most.load()) {
+      if (spare >= 0) blocks.release_spare(spare);
       const size_t before = blocks.held.size();
       for (const auto& p : parts) {
         cudaError_t e = hook();
@@ -757,11 +760,7 @@ struct Carve {
     if (spare >= 0 && blocks.spare_bytes[spare] >= bytes()) {
       block = blocks.spare[spare];
     } else {
-      if (spare >= 0) {
-        cudaFree(blocks.spare[spare]);
-        blocks.spare[spare] = nullptr;
-        blocks.spare_bytes[spare] = 0;
-      }
+      if (spare >= 0) blocks.release_spare(spare);
       const cudaError_t e = cudaMalloc(&block, bytes());
       if (e != cudaSuccess) return e;
       if (spare >= 0) {
@@ -1261,6 +1260,11 @@ extern "C" tsp_status tsp_sirt_chunked(const tsp_batch_item* items, int n_items,
         ws = nullptr;
         ws_bytes = 0;
         cudaError_t e = dev_malloc(&ws, need);
+        if (e == cudaErrorMemoryAllocation) {  // the builds' spare scratch first
+          cudaGetLastError();  // not sticky: clear it
+          scratch.release_spares();
+          e = dev_malloc(&ws, need);
+        }
         if (e != cudaSuccess) return cuda_fail(e, "tsp_sirt_chunked: workspace");
         ws_bytes = need;
       }
@@ -1277,13 +1281,13 @@ extern "C" tsp_status tsp_sirt_chunked(const tsp_batch_item* items, int n_items,
     tsp_segments s = nullptr;
     st = build_lists(items[i].grid, items[i].geom, 1, scratch, &s, stream);
     if (st == TSP_ENOMEM && !chunk.empty()) {  // no room next to the chunk: finish it, then retry alone
+      scratch.release_spares();  // (the workspace may have to be allocated now)
       st = run_chunk(first);
       if (st == TSP_OK) {
         cudaError_t e = cudaStreamSynchronize(cs);
         if (e != cudaSuccess) st = cuda_fail(e, "tsp_sirt_chunked: sync");
       }
       release();
-      scratch.release_spares();
       first = i;
       if (st == TSP_OK) st = build_lists(items[i].grid, items[i].geom, 1, scratch, &s, stream);
     }

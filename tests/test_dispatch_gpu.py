@@ -540,3 +540,37 @@ def test_build_out_of_memory_between_single_allocations(transpose, limit):
     torch.cuda.synchronize()
     assert torch.cuda.mem_get_info()[0] >= free0 - (64 << 20)
     assert tsp_device_status() == 0
+
+
+def test_chunked_workspace_after_out_of_memory():
+    """The SIRT workspace fails to be allocated once while the builds' scratch
+    is kept for the next item: the driver gives that back and tries again, and
+    every item ends as without the failure."""
+    import ctypes
+    from paper_2608_16960_gb300._lib import load
+    from paper_2608_16960_gb300.projector import Segments, sirt_chunked, tsp_device_status
+    L = load()
+    count = ctypes.c_int64()
+    items, per_item = [], 0
+    for k in range(2):
+        grid, _ = _grid((8 + 2 * k, 6 + k, 12 + 4 * k))
+        geom = _geometry("cone", 2, (24, 24))
+        y = torch.tensor(synth.uniform_volume(geom.det_shape, 7 + k, 0.5, 1.0), device="cuda")
+        items.append((grid, geom, y))
+        L.tsp_debug_allocation_count(ctypes.byref(count))
+        n0 = count.value
+        Segments(grid, geom)
+        L.tsp_debug_allocation_count(ctypes.byref(count))
+        per_item += count.value - n0
+    runs = []
+    try:
+        for fail_at in (-1, per_item):
+            xs = [(g, m, y, torch.zeros(g.shape, device="cuda")) for g, m, y in items]
+            L.tsp_debug_fail_allocation(fail_at)
+            sirt_chunked(xs, 3, budget_bytes=1 << 40)
+            runs.append([x[3] for x in xs])
+    finally:
+        L.tsp_debug_fail_allocation(-1)
+    for a, b in zip(*runs):
+        assert torch.equal(a, b)
+    assert tsp_device_status() == 0
