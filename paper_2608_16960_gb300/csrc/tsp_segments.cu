@@ -7,6 +7,7 @@
 // and multiply an input gathered from L2 (the volume, or the detector values),
 // summed per output row in registers.
 #include <atomic>
+#include <cstring>
 #include <limits>
 
 #include "tsp_kernels.cuh"
@@ -383,6 +384,32 @@ __global__ void __launch_bounds__(256) interleave_kernel(const int64_t* __restri
       const int64_t to = q + __popc(m & below);
       idx[to] = idx_in[from + k];
       len[to] = len_in[from + k];
+    }
+    q += __popc(m);
+  }
+}
+
+// The entries of the rays a .. z - 1 ray after ray (to: their offsets, from ray
+// a's) out of the interleaved rows from p0 (a multiple of 32) on.
+__global__ void __launch_bounds__(256) export_kernel(const int64_t* __restrict__ off, int64_t p0, int64_t n_rows,
+                                                     RowOrder order, const uint32_t* __restrict__ idx,
+                                                     const float* __restrict__ len, int64_t a, int64_t z,
+                                                     const int64_t* __restrict__ to, uint32_t* __restrict__ idx_out,
+                                                     float* __restrict__ len_out) {
+  const int64_t row = p0 + int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const unsigned below = (1u << (threadIdx.x & 31)) - 1u;
+  const int64_t o0 = off[min(row, n_rows)], o1 = off[min(row + 1, n_rows)];
+  const int n = int(o1 - o0), most = __reduce_max_sync(0xffffffffu, n);
+  const int64_t ray = row < n_rows ? order.ray(row) : -1;
+  const bool mine = ray >= a && ray < z;
+  const int64_t out = mine ? to[ray - a] - to[0] : 0;
+  int64_t q = __shfl_sync(0xffffffffu, o0, 0);
+  for (int k = 0; k < most; ++k) {
+    const unsigned m = __ballot_sync(0xffffffffu, k < n);
+    if (mine && k < n) {
+      const int64_t at = q + __popc(m & below);
+      idx_out[out + k] = idx[at];
+      len_out[out + k] = len[at];
     }
     q += __popc(m);
   }
@@ -1068,6 +1095,11 @@ extern "C" tsp_status tsp_segments_info(tsp_segments s, int64_t* n_rays, int64_t
   return TSP_OK;
 }
 
+// The lists to the host ray after ray, in pieces of whole rays through device
+// buffers of 40 MB (less where there is less); a host loop over the entries takes
+// ten times as long. The host's pages are touched first: several copies into
+// pages that are not mapped yet took as long as that loop (106 M segments: 640 ms;
+// 49 now, 56 in one copy per array when the lists lay ray after ray).
 extern "C" tsp_status tsp_segments_export(tsp_segments s, int64_t* ray_off, uint32_t* vox, float* len) {
   if (!s) return fail(TSP_EINVAL, "tsp_segments_export: NULL handle");
   tsp_status st = check_device(s->device);
@@ -1076,32 +1108,63 @@ extern "C" tsp_status tsp_segments_export(tsp_segments s, int64_t* ray_off, uint
   const int64_t n = s->n_rays;
   std::vector<int64_t> off(size_t(n + 1)), to(size_t(n + 1), 0);  // of the rows, of the rays
   TSP_CUDA(cudaMemcpy(off.data(), s->fwd.off, sizeof(int64_t) * off.size(), cudaMemcpyDeviceToHost));
-  for (int64_t p = 0; p < n; ++p) to[size_t(s->order.ray(p) + 1)] = off[size_t(p + 1)] - off[size_t(p)];
-  for (int64_t r = 0; r < n; ++r) to[size_t(r + 1)] += to[size_t(r)];
-  if (ray_off) std::copy(to.begin(), to.end(), ray_off);
-  const size_t S = size_t(s->n_segs);
-  if (S == 0 || (!vox && !len)) return TSP_OK;
-  std::vector<uint32_t> iv(vox ? S : 0);
-  std::vector<float> lv(len ? S : 0);
-  if (vox) TSP_CUDA(cudaMemcpy(iv.data(), s->fwd.idx, sizeof(uint32_t) * S, cudaMemcpyDeviceToHost));
-  if (len) TSP_CUDA(cudaMemcpy(lv.data(), s->fwd.len, sizeof(float) * S, cudaMemcpyDeviceToHost));
-  size_t q = 0;
-  for (int64_t p0 = 0; p0 < n; p0 += 32) {  // slices back to rays
-    const int64_t p1 = std::min(p0 + 32, n);
-    bool any = true;
-    for (int64_t k = 0; any; ++k) {
-      any = false;
-      for (int64_t p = p0; p < p1; ++p) {
-        if (off[size_t(p)] + k >= off[size_t(p + 1)]) continue;
-        any = true;
-        const size_t at = size_t(to[size_t(s->order.ray(p))] + k);
-        if (vox) vox[at] = iv[q];
-        if (len) len[at] = lv[q];
-        ++q;
-      }
-    }
+  const RowOrder order = s->order;
+  if (order.W == 0) {
+    to = off;
+  } else {
+    int64_t p = 0;
+    for (int64_t r0 = 0; r0 < n; r0 += int64_t(order.H) * order.W)  // views, bands, columns, rows of a band
+      for (int i0 = 0; i0 < order.H; i0 += 4)
+        for (int64_t col = 0; col < order.W; ++col)
+          for (int i = i0; i < std::min(i0 + 4, order.H); ++i, ++p)
+            to[size_t(r0 + int64_t(i) * order.W + col + 1)] = off[size_t(p + 1)] - off[size_t(p)];
+    for (int64_t r = 0; r < n; ++r) to[size_t(r + 1)] += to[size_t(r)];
   }
-  return TSP_OK;
+  if (ray_off) std::copy(to.begin(), to.end(), ray_off);
+  if (s->n_segs == 0 || (!vox && !len)) return TSP_OK;
+  if (vox) std::memset(vox, 0, sizeof(uint32_t) * size_t(s->n_segs));
+  if (len) std::memset(len, 0, sizeof(float) * size_t(s->n_segs));
+  int64_t widest = 0;
+  for (int64_t r = 0; r < n; ++r) widest = std::max(widest, to[size_t(r + 1)] - to[size_t(r)]);
+  int64_t most = std::max(widest, std::min(s->n_segs, int64_t(1) << 22)), rays = std::min(n, int64_t(1) << 20);
+  char* stage = nullptr;
+  for (;;) {  // [rays + 1] offsets, [most] columns, [most] lengths
+    const cudaError_t e = cudaMalloc(&stage, size_t(8 * (rays + 1) + 8 * most));
+    if (e == cudaSuccess) break;
+    if (most / 2 < std::max(widest, int64_t(1) << 16)) return cuda_fail(e, "tsp_segments_export: staging");
+    cudaGetLastError();  // not sticky: clear it
+    most /= 2;
+    rays = std::max<int64_t>(1, rays / 2);
+  }
+  int64_t* const d_to = reinterpret_cast<int64_t*>(stage);
+  uint32_t* const d_vox = reinterpret_cast<uint32_t*>(stage + 8 * (rays + 1));
+  float* const d_len = reinterpret_cast<float*>(d_vox + most);
+  cudaError_t e = cudaSuccess;
+  for (int64_t a = 0, z; a < n && e == cudaSuccess; a = z) {
+    for (z = a + 1; z < n && z - a < rays && to[size_t(z + 1)] - to[size_t(a)] <= most;) ++z;
+    const size_t m = size_t(to[size_t(z)] - to[size_t(a)]);
+    if (m == 0) continue;
+    // the rows of these rays lie in their bands (their ranges of rows and of rays are the same)
+    int64_t p0 = a, p1 = z;
+    if (order.W > 0) {
+      const int64_t plane = int64_t(order.H) * order.W, band = 4 * int64_t(order.W);
+      p0 = a / plane * plane + a % plane / band * band;
+      const int64_t v = (z - 1) / plane * plane;
+      p1 = v + std::min(plane, ((z - 1 - v) / band + 1) * band);
+    }
+    p0 = p0 / 32 * 32;
+    e = cudaMemcpy(d_to, to.data() + a, sizeof(int64_t) * size_t(z - a + 1), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) break;
+    export_kernel<<<unsigned((p1 - p0 + 255) / 256), 256>>>(s->fwd.off, p0, n, order, s->fwd.idx, s->fwd.len, a, z,
+                                                           d_to, d_vox, d_len);
+    e = cudaGetLastError();
+    if (e == cudaSuccess && vox)
+      e = cudaMemcpy(vox + to[size_t(a)], d_vox, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess && len)
+      e = cudaMemcpy(len + to[size_t(a)], d_len, sizeof(float) * m, cudaMemcpyDeviceToHost);
+  }
+  cudaFree(stage);
+  return e == cudaSuccess ? TSP_OK : cuda_fail(e, "tsp_segments_export");
 }
 
 extern "C" tsp_status tsp_segments_export_transposed(tsp_segments s, int64_t* vox_off, uint32_t* ray, float* len) {
