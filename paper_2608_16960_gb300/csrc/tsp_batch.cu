@@ -309,6 +309,9 @@ extern "C" tsp_status tsp_batch_create(const tsp_batch_item* items, int n_items,
     delete b;
     return cuda_fail(e, "cudaGetDevice");
   }
+  double all_rays = 0.0;
+  for (int i = 0; i < n_items; ++i)
+    if (items[i].geom) all_rays += double(items[i].geom->n_rays);
   int64_t most_rays = -1;
   tsp_launch lead = default_launch();
   for (int i = 0; i < n_items; ++i) {
@@ -318,7 +321,8 @@ extern "C" tsp_status tsp_batch_create(const tsp_batch_item* items, int n_items,
       delete b;
       return st;
     }
-    tsp_launch lf = preferred_launch(it.grid, it.geom, false), la = preferred_launch(it.grid, it.geom, true);
+    const double share = all_rays / double(std::max<int64_t>(1, it.geom->n_rays));
+    tsp_launch lf = preferred_launch(it.grid, it.geom, false), la = preferred_launch(it.grid, it.geom, true, 1, share);
     if (it.geom->n_rays > most_rays) {
       most_rays = it.geom->n_rays;
       lead = lf;

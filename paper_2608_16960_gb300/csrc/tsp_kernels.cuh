@@ -423,12 +423,27 @@ inline double pixels_per_voxel(const tsp_grid_s* grid, const tsp_geom_s* geom) {
 // views of 256^2 on 100 x 60 x 120) 1792 / 1431 / 1516, 6.9 pixels 1400 /
 // 1073 / 1103, 10.4 pixels 2641 / 1659 / 1374, 21 pixels 2359 / 1280 / 488;
 // three values at 3 pixels 354 / 304 / 287, at 5.2 pixels 692 / 490 / 401.
-// Below 65536 rays the walk's latency hides the queueing.
-inline tsp_launch preferred_launch(const tsp_grid_s* grid, const tsp_geom_s* geom, bool adjoint, int values = 1) {
+// Where the rays are few or the grid is fine, the walk's latency hides the
+// queueing and combining lanes only lengthens it: the line lies at rays times
+// crossings per voxel, n_rays^2 (N_r + N_e + N_a) / voxels, of 18.5 M (one add /
+// combined; 66 k to 202 k rays of 1 to 8 views): 11 M 111 / 121, 13 M 61 / 69, 16 M
+// 170 / 168, 18 M 102 / 108, 18.5 M 106 / 104, 19 M 70 / 69, 24 M 81 / 70, 31 M 93 /
+// 87, 33 M 85 / 69; with three values at 12 M: 8 M 102 / 124, 11 M 189 / 199, 11.5 M
+// 109 / 119, 13 M 107 / 99, 15 M 130 / 126, 18 M 183 / 160. `share` multiplies it:
+// a view's rays are alone in their volume where the object changes (1 / views;
+// 8 M 74 / 80, 15 M 108 / 109, 27 M 120 / 112), the rays of a batch are under way
+// together (all rays / the item's; 47 M 603 / 564). Below 65536 rays none are
+// combined: of 4 k to 63 k rays those on fine grids would lose (109 / 130, 118 /
+// 144), those on coarse ones gain (78 / 51, 76 / 29).
+inline tsp_launch preferred_launch(const tsp_grid_s* grid, const tsp_geom_s* geom, bool adjoint, int values = 1,
+                                   double share = 1.0) {
   tsp_launch f, a;
   if (tuned_launch(grid, geom, &f, &a)) return adjoint ? a : f;
   tsp_launch l = default_launch();
-  if (adjoint && geom->n_rays >= 65536 && pixels_per_voxel(grid, geom) >= (values > 1 ? 2.5 : 4.0)) l.scatter = 1;
+  if (adjoint && geom->n_rays >= 65536 && pixels_per_voxel(grid, geom) >= (values > 1 ? 2.5 : 4.0)) {
+    const double rays = double(geom->n_rays), crossings = rays * (grid->Nr + grid->Ne + grid->Na) / double(grid->voxels());
+    if (share * rays * crossings >= (values > 1 ? 12e6 : 18.5e6)) l.scatter = 1;
+  }
   return l;
 }
 

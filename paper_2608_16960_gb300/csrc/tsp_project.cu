@@ -206,9 +206,9 @@ extern "C" tsp_status tsp_adjoint_dynamic(tsp_grid grid, tsp_geom geom, const fl
   TSP_RANGE("tsp_adjoint_dynamic");
   tsp_status st = check_trace_args(grid, geom, y, rho, 1, nullptr, "tsp_adjoint_dynamic");
   if (st != TSP_OK) return st;
-  const tsp_launch l = preferred_launch(grid, geom, true);
-  const int64_t V = grid->voxels();
   const int nv = std::max(1, geom->n_views);
+  const tsp_launch l = preferred_launch(grid, geom, true, 1, 1.0 / nv);
+  const int64_t V = grid->voxels();
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   if (!accumulate) TSP_CUDA(cudaMemsetAsync(rho, 0, sizeof(float) * size_t(V) * nv, cs));
   auto go = [&](auto op) {

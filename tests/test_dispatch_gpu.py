@@ -601,3 +601,40 @@ def test_export_of_many_rays(kind, n_views, det):
     ref = tsp_forward(grid, geom, rho).double().cpu().numpy().reshape(-1)
     assert np.abs(y - ref).max() <= 1e-5 * ref.max()
     assert t <= max(3e-9 * len(vox), 0.02), (t, len(vox))
+
+
+@pytest.mark.parametrize("shape,n_views,det,dynamic", [((60, 36, 72), 1, 257, False), ((80, 45, 90), 1, 300, False),
+                                                      ((40, 30, 60), 4, 181, True)])
+def test_scatters_of_few_rays_are_not_combined_at_a_loss(shape, n_views, det, dynamic):
+    """Wide voxels, but few rays on a fine grid: the untuned adjoint takes no
+    longer than one add per segment (5% for the clock; combined it takes 8 to 23% longer)."""
+    from paper_2608_16960_gb300.projector import (tsp_adjoint, tsp_adjoint_dynamic, tsp_autotune_clear,
+                                                  tsp_autotune_store)
+    grid, _ = _grid(shape)
+    geom = _geometry("cone", n_views, (det, det))
+    y = torch.rand(geom.det_shape, device="cuda")
+    out = torch.empty(((n_views,) if dynamic else ()) + grid.shape, device="cuda")
+    call = (lambda: tsp_adjoint_dynamic(grid, geom, y, out)) if dynamic else (lambda: tsp_adjoint(grid, geom, y, out))
+
+    def time():
+        for _ in range(10):
+            call()
+        torch.cuda.synchronize()
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(50):
+            call()
+        b.record()
+        b.synchronize()
+        return a.elapsed_time(b)
+
+    untuned, plain = [], []
+    try:
+        for _ in range(3):
+            tsp_autotune_clear()
+            untuned.append(time())
+            tsp_autotune_store(grid, geom, (128, 8, 0), (128, 8, 0))
+            plain.append(time())
+    finally:
+        tsp_autotune_clear()
+    assert min(untuned) <= 1.05 * min(plain), (untuned, plain)
