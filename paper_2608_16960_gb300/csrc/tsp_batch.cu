@@ -9,7 +9,8 @@
 // way. The whole schedule (weights + n_iter iterations) is captured once into
 // a CUDA graph and replayed with a single graph launch. Per instance, the
 // warp tile and the scatter strategy come from the autotuner's size-class
-// cache (tsp_autotune), the block size from the instance with the most rays.
+// cache (tsp_autotune), or without an entry there from the rules of
+// preferred_launch; the block size comes from the instance with the most rays.
 #include <algorithm>
 #include <vector>
 
@@ -251,7 +252,7 @@ size_t batch_ws_bytes(const tsp_batch_s* b, int n_stage_counters) {
          align256(sizeof(unsigned long long) * size_t(n_stage_counters));
 }
 
-int counters_for(int n_iter) { return 3 + 3 * n_iter; }
+int counters_for(int n_iter) { return 2 + 3 * n_iter; }
 
 // Enqueue the whole batched SIRT schedule on st (capturable).
 tsp_status enqueue_batch(tsp_batch b, int n_iter, int flags, void* ws, cudaStream_t st) {

@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(256) slice_forward_kernel(const int64_t* __res
 template <int G, int U, int NB, bool EPI>
 __global__ void __launch_bounds__(256) row_group_kernel(const int64_t* __restrict__ off,
                                                         const uint32_t* __restrict__ idx,
-                                                        const float* __restrict__ len, int64_t S, int64_t n_rows,
+                                                        const float* __restrict__ len, int64_t n_rows,
                                                         uint32_t col_max, const float* __restrict__ src,
                                                         int64_t src_stride, float* __restrict__ dst,
                                                         int64_t dst_stride, int nb, int flag,
@@ -651,13 +651,13 @@ void row_groups(const SegList& l, const float* src, float* dst, int k, int flag,
   const unsigned blocks = unsigned((l.n_rows * G + 255) / 256);
   const uint32_t cm = uint32_t(l.n_cols - 1);
   if (C)
-    row_group_kernel<G, U, 1, true><<<blocks, 256, 0, st>>>(l.off, l.idx, l.len, l.S, l.n_rows, cm, src, l.n_cols, dst,
+    row_group_kernel<G, U, 1, true><<<blocks, 256, 0, st>>>(l.off, l.idx, l.len, l.n_rows, cm, src, l.n_cols, dst,
                                                             l.n_rows, 1, flag, C);
   else if (k == 1)
-    row_group_kernel<G, U, 1, false><<<blocks, 256, 0, st>>>(l.off, l.idx, l.len, l.S, l.n_rows, cm, src, l.n_cols,
+    row_group_kernel<G, U, 1, false><<<blocks, 256, 0, st>>>(l.off, l.idx, l.len, l.n_rows, cm, src, l.n_cols,
                                                              dst, l.n_rows, 1, flag, nullptr);
   else
-    row_group_kernel<G, U, 4, false><<<blocks, 256, 0, st>>>(l.off, l.idx, l.len, l.S, l.n_rows, cm, src, l.n_cols,
+    row_group_kernel<G, U, 4, false><<<blocks, 256, 0, st>>>(l.off, l.idx, l.len, l.n_rows, cm, src, l.n_cols,
                                                              dst, l.n_rows, k, flag, nullptr);
 }
 
