@@ -1163,7 +1163,8 @@ inline size_t thin_smem(int Na, int mode) {
 }
 
 // f = hi + mid + lo, each a bf16 (the bits of its upper half), exactly: the
-// three bytes of its significand. Infinities and NaN stay in hi.
+// three bytes of its significand. An infinity or a NaN is all three: beside an
+// infinite hi, zeros would make NaN of its products with infinities.
 struct Split3 {
   uint32_t p[3];  // lo, mid, hi
 };
@@ -1172,10 +1173,10 @@ __device__ __forceinline__ Split3 split3(float f) {
   const bool finite = (b & 0x7f800000u) != 0x7f800000u;
   uint32_t hi = b & 0xffff0000u;
   if (f != f) hi |= 0x00400000u;
-  const float r = finite ? f - __uint_as_float(hi) : 0.0f;
-  const uint32_t mid = __float_as_uint(r) & 0xffff0000u;
+  const float r = f - __uint_as_float(hi);
+  const uint32_t mid = finite ? __float_as_uint(r) & 0xffff0000u : hi;
   Split3 o;
-  o.p[0] = __float_as_uint(r - __uint_as_float(mid)) >> 16;
+  o.p[0] = (finite ? __float_as_uint(r - __uint_as_float(mid)) : hi) >> 16;
   o.p[1] = mid >> 16;
   o.p[2] = hi >> 16;
   return o;

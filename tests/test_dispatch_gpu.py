@@ -638,3 +638,23 @@ def test_scatters_of_few_rays_are_not_combined_at_a_loss(shape, n_views, det, dy
     finally:
         tsp_autotune_clear()
     assert min(untuned) <= 1.05 * min(plain), (untuned, plain)
+
+
+def test_network_gradients_of_an_infinite_input():
+    """One infinite voxel, everything positive, the reach of all layers inside
+    the grid: activations, output and gradients around it are +inf, so every
+    weight's and bias's gradient is a sum of positive terms of which some are
+    infinite: +inf, not NaN."""
+    from oracle import net as onet
+    from paper_2608_16960_gb300.model import WarmStartNet
+    shape = (32, 32, 32)
+    net = WarmStartNet(shape, 1)
+    params = [(np.full_like(w, 1.0 / 1024), np.full_like(b, 0.01)) for w, b in onet.init_params(3)]
+    net.set_params(np.concatenate([np.concatenate([w.ravel(), b.ravel()]) for w, b in params]))
+    a = torch.full((1,) + shape, 0.5, device="cuda")
+    a[0, 16, 16, 16] = float("inf")
+    loss = net.loss_grad(a, torch.zeros_like(a))
+    got = net.get_grads()
+    assert loss == np.inf
+    for k, (off, sh) in enumerate(net.layout()):
+        assert (got[off:off + int(np.prod(sh))] == np.inf).all(), k
