@@ -658,3 +658,78 @@ def test_network_gradients_of_an_infinite_input():
     assert loss == np.inf
     for k, (off, sh) in enumerate(net.layout()):
         assert (got[off:off + int(np.prod(sh))] == np.inf).all(), k
+
+
+@pytest.mark.parametrize("na", [32, 64, 96, 128, 160, 192])
+def test_network_gradients_across_the_azimuth_wrap(na):
+    """Input and gradient at azimuths 0 and N_a - 1 alone: the taps da = -1 and
+    +1 of the weight gradients then consist of the wrapped terms, which the ring
+    slots' copies hold by a patch of their own. Layers that pass their input
+    through (zero weights; biases of 2^-20, which open the masks and are lost in
+    bfloat16 beside an input), powers of two for operands: every product is
+    exact, and the sums of at most 64 terms are held to 2^-16 of their
+    magnitudes' (64 additions cut off at 2^-23 each, four times over)."""
+    from oracle import net as onet
+    from paper_2608_16960_gb300.model import WarmStartNet
+    shape, batch = (4, 8, na), 1
+    net = WarmStartNet(shape, batch)
+    params = [(np.zeros_like(w), np.full_like(b, 2.0 ** -20)) for w, b in onet.init_params(3)]
+    params[0][0][13, :, 0] = 2.0 ** -(np.arange(32) % 4)
+    params[0][1][:] = 0.0
+    params[5][0][13, 0, :] = 2.0 ** -(np.arange(32) % 3)
+    params[5][1][:] = 0.0
+    net.set_params(np.concatenate([np.concatenate([w.ravel(), b.ravel()]) for w, b in params]))
+    rng = np.random.default_rng(4)
+    a = np.zeros((batch,) + shape, np.float32)
+    a[..., [0, na - 1]] = 2.0 ** rng.integers(-2, 3, (batch,) + shape[:2] + (2,))
+    # the target that leaves a gradient of powers of two there and none elsewhere
+    out = net.forward(torch.tensor(a, device="cuda")).cpu().numpy()
+    g = np.zeros_like(a)
+    g[..., [0, na - 1]] = 2.0 ** rng.integers(-2, 3, (batch,) + shape[:2] + (2,))
+    net.loss_grad(torch.tensor(a, device="cuda"), torch.tensor(out - g, device="cuda"))
+    got = net.get_grads()
+    x0 = a[..., None].astype(np.float64) * params[0][0][13, :, 0]
+    mean = float(torch.tensor(np.float32(2.0 / a.size)).bfloat16())
+    gz = mean * g[..., None].astype(np.float64) * params[5][0][13, 0]
+
+    def shift(x, o):
+        z = np.roll(x, (-o[0], -o[1], -o[2]), (1, 2, 3))
+        for d in (0, 1):
+            if o[d]:
+                idx = [slice(None)] * z.ndim
+                idx[d + 1] = -1 if o[d] > 0 else 0
+                z[tuple(idx)] = 0.0
+        return z
+
+    for layer in (1, 2, 3, 4):
+        off, sh = net.layout()[2 * layer]
+        dw = got[off:off + 27 * 32 * 32].reshape(27, 32, 32)
+        for tap in range(27):
+            o = (tap // 9 - 1, tap // 3 % 3 - 1, tap % 3 - 1)
+            xs = shift(np.where(x0 > 0.0, x0, (layer - 1) * 2.0 ** -20), o).reshape(-1, 32)
+            ref = gz.reshape(-1, 32).T @ xs
+            assert (ref > 2.0 ** -12 * gz.max()).all()
+            assert (np.abs(dw[tap] - ref) <= 2.0 ** -16 * ref).all(), (layer, tap, np.abs(dw[tap] / ref - 1.0).max())
+
+
+def test_lists_of_one_handle_on_two_streams():
+    """Forward and adjoint calls on one handle enqueued on two streams at once
+    share nothing but the lists: each result is that of the call by itself."""
+    from paper_2608_16960_gb300.projector import Segments
+    grid, _ = _grid((30, 24, 48))
+    geom = _geometry("cone", 8, (128, 128))
+    segs = Segments(grid, geom)
+    rho = [torch.tensor(synth.uniform_volume((b,) + grid.shape, 3 + b, 0.1, 1.0), device="cuda") for b in (1, 3)]
+    w = [torch.tensor(synth.uniform_volume((b,) + geom.det_shape, 5 + b, 0.1, 1.0), device="cuda") for b in (1, 3)]
+    alone = [(segs.forward(r), segs.adjoint(v)) for r, v in zip(rho, w)]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    got = [[], []]
+    for _ in range(20):
+        for k, st in enumerate(streams):
+            with torch.cuda.stream(st):
+                got[k].append((segs.forward(rho[k]), segs.adjoint(w[k])))
+    torch.cuda.synchronize()
+    for k in range(2):
+        for y, g in got[k]:
+            assert torch.equal(y, alone[k][0]) and torch.equal(g, alone[k][1])
