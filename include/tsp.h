@@ -188,8 +188,9 @@ tsp_status tsp_count_segments(tsp_grid grid, tsp_geom geom, int* counts, void* s
 typedef struct tsp_segments_s* tsp_segments;
 
 /*
- * tsp_segments_build - traverses every ray of geom twice (count, then fill)
- * and builds the lists on grid's device. Synchronises `stream` (it reads the
+ * tsp_segments_build - traverses every ray of geom twice (count, then fill;
+ * lists filled in pieces again for each) and builds the lists on grid's device.
+ * Synchronises `stream` (it reads the
  * total segment count back to size the lists). *out receives the handle, or
  * NULL on error. TSP_ENOMEM/TSP_ECUDA on allocation or launch failure.
  */
@@ -427,8 +428,9 @@ void tsp_batch_destroy(tsp_batch batch);
  * for a chunk of consecutive items that fits budget_bytes (0: 80% of the
  * free device memory), every iteration of those items runs from them, and
  * they are freed before the next chunk (an item whose lists do not fit next
- * to the chunk starts a new one). Synchronous (the builds read segment
- * counts back). n_chunks, peak_bytes (either may be NULL) receive the
+ * to the chunk starts a new one). budget_bytes and peak_bytes count the lists;
+ * the builds' temporary memory (tsp_segments_build) and one SIRT workspace come
+ * beside them. Synchronous (the builds read segment counts back). n_chunks, peak_bytes (either may be NULL) receive the
  * number of chunks and the largest list memory held at once.
  * TSP_ENOMEM if one item's lists alone do not fit.
  */

@@ -106,8 +106,9 @@ __device__ __forceinline__ void cp_async16_zfill(void* smem, const void* gmem, u
 // (tcgen05.ld 32x32b) while the tensor cores work on the next.
 //
 // Batch 8 of 64 x 48 x 96 on GB300: output layer 138 us, bound by the MMAs
-// (about 120 cycles each, 80 with N = 32: most of it the window's read from
-// shared memory, so fewer, wider MMAs win); forward layer 168 and dgrad 267,
+// (about 100 cycles each over the 80 steps of the longest CTA, 67 with N = 32:
+// most of it the window's read from shared memory, so fewer, wider MMAs win; the
+// CTAs' mean is 67 steps); forward layer 168 and dgrad 267,
 // bound by the epilogue (157 and 249 with half of the MMAs left out). With the
 // operands read back one step ahead in registers (56 / 224 registers a thread
 // by setmaxnreg) 169 and 262.
@@ -684,7 +685,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv32_tc_kernel(const __grid_c
 //
 // Measured at batch 8, 64 x 48 x 96 on GB300: 435 us a layer before (N = 32
 // with one MMA per azimuth tap over 16-byte channel planes, all nine rows
-// loaded again for every output row), 189 us now. It is bound by the tensor
+// loaded again for every output row), 195 us now. It is bound by the tensor
 // cores (about 130 cycles per MMA): fewer bytes loaded or longer rings change
 // nothing, a third of the MMAs takes 139 us. Issued by one elected lane: with
 // elect.sync around every MMA the same kernel took 243 us.
