@@ -437,12 +437,14 @@ def test_lists_of_a_large_grid_that_few_rays_meet(fov, empty):
     grid, _ = _grid((250, 256, 1000))
     pos = synth.circular_orbit(1, 60.0, incline_deg=20.0, phase=0.3)
     geom = Geometry.cone(pos, (8, 8), fov, look_at=2.0 * pos if empty else None)
-    Segments(grid, geom)
-    torch.cuda.synchronize()
-    t0 = time.perf_counter()
-    s = Segments(grid, geom)
-    torch.cuda.synchronize()
-    t = time.perf_counter() - t0
+    ts = []
+    for _ in range(4):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        s = Segments(grid, geom)
+        torch.cuda.synchronize()
+        ts.append(time.perf_counter() - t0)
+    t = min(ts)
     off, vox, _ = s.export()
     assert (off[-1] == 0) == empty
     voff = s.export_transposed()[0]
